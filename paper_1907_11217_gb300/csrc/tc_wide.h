@@ -714,8 +714,16 @@ __global__ void __launch_bounds__(kWideThreads, 1)
           scale8(c);
           if (n0 + c < a.N) {
             uint8_t *buf = buf0 + (c & 8) * 256;
-            // the store before the last has read this buffer
-            if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+            // the last store that used this buffer has read it: the one before
+            // the last within a tile; a tile starts over at the first buffer,
+            // which the last store of the tile before may also have used (an odd
+            // number of chunks), so there every store has
+            if (lane == 0) {
+              if (c == 0)
+                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+              else
+                asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+            }
             __syncwarp();
 #pragma unroll
             for (int j = 0; j < 4; j++)
