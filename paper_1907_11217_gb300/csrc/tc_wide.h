@@ -709,17 +709,22 @@ __global__ void __launch_bounds__(kWideThreads, 1)
         }
       } else if (a.tma_store) {
         const int y = (int)(d.z * a.M + d.row0 + q * 32);
+        // chunks use the two buffers in turn and a tile starts over at the
+        // first; a warp's last chunk of a tile used the first as well only with
+        // an odd number of chunks in a row of C (waiting there in every tile
+        // costs what the stores of short K overlap: FP16 b256 M4096 N512 K32
+        // 1024 -> 1081 us, so 1030)
+        const bool odd = ((a.N + 7) >> 3) & 1;
 #pragma unroll
         for (int c = 0; c < EC; c += 8) {
           scale8(c);
           if (n0 + c < a.N) {
             uint8_t *buf = buf0 + (c & 8) * 256;
-            // the last store that used this buffer has read it: the one before
-            // the last within a tile; a tile starts over at the first buffer,
-            // which the last store of the tile before may also have used (an odd
-            // number of chunks), so there every store has
+            // the store before the last has read this buffer (the first chunk of
+            // a tile: every store has, where the last store of the tile before
+            // may have used this buffer too)
             if (lane == 0) {
-              if (c == 0)
+              if (c == 0 && odd)
                 asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
               else
                 asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
