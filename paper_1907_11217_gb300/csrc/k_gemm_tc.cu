@@ -430,6 +430,15 @@ __device__ __forceinline__ int64_t scatter_bits(int64_t v, int n, const int8_t *
   return o;
 }
 
+// A store of C, as streaming data (evict first) or with the normal priority.
+template <typename T>
+__device__ __forceinline__ void store_c(T *p, T v, bool streaming) {
+  if (streaming)
+    __stcs(p, v);
+  else
+    *p = v;
+}
+
 // Accumulation range: the tensor cores sum at most kFoldK real K values (of
 // each of the three products) in one TMEM accumulator. Their FP32
 // accumulation rounds toward zero: on GB300 a product summed over K real
@@ -485,6 +494,29 @@ struct TcSmem {
   // an exponent entry, or its barrier's next phase, that the epilogue has yet
   // to read
   static_assert(XR == 0 || XR >= ASLOTS + NBUF + 1, "exponent ring deep enough");
+};
+
+// L2 prefetch of A: a second cursor walks the loader's k-blocks a.prefetch
+// ahead of its loads, so that a load finds its A tile in L2.
+template <typename Tile>
+struct ACursor {
+  int64_t t;
+  bool on;
+  int kb = -1;
+  Tile d{};
+  __device__ ACursor(int64_t walker, bool on_) : t(walker), on(on_) {}
+  // to the next k-block (kb of tile d); false when there is none, or when off
+  template <typename Decode>
+  __device__ __forceinline__ bool next(int64_t n_tiles, int64_t n_walkers, const Decode &decode) {
+    if (!on) return false;
+    if (kb < 0 || ++kb >= d.kb1) {
+      if (kb >= 0) t += n_walkers;
+      if (t >= n_tiles) return on = false;
+      d = decode(t);
+      kb = d.kb0;
+    }
+    return true;
+  }
 };
 
 // Persistent: each CTA walks tiles blockIdx.x, blockIdx.x + gridDim.x, ...
@@ -628,25 +660,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool prepared = false;  // the preparation of B has ended
       uint32_t g = 0;  // k-blocks issued by this CTA
       bool ok = true;
-      // L2 prefetch of A: a second cursor walks the same k-blocks a.prefetch
-      // ahead of the loads, so that a load finds its A tile in L2
-      int64_t pt = walker;
-      int pkb = -1;
-      Tile pd{};
-      bool pf = a.prefetch > 0;
+      ACursor<Tile> pc{walker, a.prefetch > 0};
       auto prefetch_next = [&]() {
-        if (!pf) return;
-        if (pkb < 0 || ++pkb >= pd.kb1) {
-          if (pkb >= 0) pt += n_walkers;
-          if (pt >= n_tiles) {
-            pf = false;
-            return;
-          }
-          pd = decode(pt);
-          pkb = pd.kb0;
-        }
+        if (!pc.next(n_tiles, n_walkers, decode)) return;
 #pragma unroll
-        for (int h = 0; h < stage_k<MODE>() / 32; h++) tma_prefetch_2d(&tmA, pkb * stage_k<MODE>() + 32 * h, pd.rowA);
+        for (int h = 0; h < stage_k<MODE>() / 32; h++) tma_prefetch_2d(&tmA, pc.kb * stage_k<MODE>() + 32 * h, pc.d.rowA);
       };
       for (int i = 0; i < a.prefetch; i++) prefetch_next();
       for (int64_t t = walker; t < n_tiles && ok; t += n_walkers) {
@@ -1482,12 +1500,12 @@ cudaError_t run_tc(const CUtensorMap &ta, const CUtensorMap &tbh, const CUtensor
 }
 
 // Wide tiles: one CTA (or half a pair, CG = 2) per SM, as run_tc.
-template <int MODE, int CG>
+template <int MODE, int CG, bool SET>
 cudaError_t run_wide(const CUtensorMap &ta, const CUtensorMap &tbh, const CUtensorMap &tbl, const CUtensorMap &tc,
                      const TcArgs &args, int64_t n_tiles, cudaStream_t s) {
   using L = WideSmem<MODE, CG>;
   static_assert(L::TOTAL <= 227 * 1024 && L::TOTAL > 114 * 1024, "one CTA per SM");
-  auto kernel = tc_wide_kernel<MODE, CG>;
+  auto kernel = tc_wide_kernel<MODE, CG, SET>;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   cfg.blockDim = dim3(kWideThreads);
@@ -1533,6 +1551,18 @@ cudaError_t run_wide(const CUtensorMap &ta, const CUtensorMap &tbh, const CUtens
   e = cudaLaunchKernelEx(&cfg, kernel, ta, tbh, tbl, tc, args);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
+}
+
+// (SET: the launch settings are not the default ones)
+template <int MODE>
+cudaError_t dispatch_wide(int cg, const CUtensorMap &ta, const CUtensorMap &tbh, const CUtensorMap &tbl,
+                          const CUtensorMap &tc, const TcArgs &args, int64_t n_tiles, cudaStream_t s) {
+  const bool set = args.prefetch > 0 || !(args.l2_mode & 2);
+  if (cg == 2)
+    return set ? run_wide<MODE, 2, true>(ta, tbh, tbl, tc, args, n_tiles, s)
+               : run_wide<MODE, 2, false>(ta, tbh, tbl, tc, args, n_tiles, s);
+  return set ? run_wide<MODE, 1, true>(ta, tbh, tbl, tc, args, n_tiles, s)
+             : run_wide<MODE, 1, false>(ta, tbh, tbl, tc, args, n_tiles, s);
 }
 
 template <int MODE>
@@ -1759,6 +1789,7 @@ cudaError_t launch_cgemm_tc(int precision, const float2 *A, const float2 *B, flo
     if (e != cudaSuccess) return e;
     TcArgs args{};
     args.err = err;
+    args.prefetch = tc_prefetch_default();
     args.l2_mode = tc_l2_mode_default();
     args.cscale = cscale;
     args.C = C;
@@ -1790,14 +1821,9 @@ cudaError_t launch_cgemm_tc(int precision, const float2 *A, const float2 *B, flo
       if (make_map(&tcm, C, 2 * N, rowsA, 16, 32, CU_TENSOR_MAP_DATA_TYPE_FLOAT32)) args.tma_store = 1;
     }
     const int64_t n_tiles = batch * args.n_tiles_m * (int64_t)args.n_tiles_n * w.ks;
-    if (w.cg == 2)
-      e = tf32  ? run_wide<MODE_TF32, 2>(ta, tbh, tbl, tcm, args, n_tiles, s)
-          : f16 ? run_wide<MODE_F16, 2>(ta, tbh, tbl, tcm, args, n_tiles, s)
-                : run_wide<MODE_BF16, 2>(ta, tbh, tbl, tcm, args, n_tiles, s);
-    else
-      e = tf32  ? run_wide<MODE_TF32, 1>(ta, tbh, tbl, tcm, args, n_tiles, s)
-          : f16 ? run_wide<MODE_F16, 1>(ta, tbh, tbl, tcm, args, n_tiles, s)
-                : run_wide<MODE_BF16, 1>(ta, tbh, tbl, tcm, args, n_tiles, s);
+    e = tf32  ? dispatch_wide<MODE_TF32>(w.cg, ta, tbh, tbl, tcm, args, n_tiles, s)
+        : f16 ? dispatch_wide<MODE_F16>(w.cg, ta, tbh, tbl, tcm, args, n_tiles, s)
+              : dispatch_wide<MODE_BF16>(w.cg, ta, tbh, tbl, tcm, args, n_tiles, s);
     if (e != cudaSuccess || w.ks == 1) return e;
     const int64_t total = batch * M * N;
     split_reduce_kernel<<<(int)std::min<int64_t>((total + 255) / 256, 152 * 8), 256, 0, s>>>(P, C, w.ks, total, M * N,

@@ -118,7 +118,11 @@ struct WideSmem {
   static_assert((2 * AST + 2 * BST + 2 * SLOTS + 2 * NACC + 2 + XR) * 8 + 16 <= BARS, "barriers and flags fit in BARS");
 };
 
-template <int MODE, int CG>
+// SET: with the launch settings (TcArgs::prefetch, bit 1 of TcArgs::l2_mode). An
+// instance of its own: as arguments of one kernel they cost products that leave
+// them at their defaults registers and branches of the loading and storing warps
+// (FP16 b256 M4096 N512 K32 1030 -> 1084 us, TF32 b64 M4096 N1024 K64 489 -> 527).
+template <int MODE, int CG, bool SET>
 __global__ void __launch_bounds__(kWideThreads, 1)
     tc_wide_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmBh,
                    const __grid_constant__ CUtensorMap tmBl, const __grid_constant__ CUtensorMap tmC, TcArgs a) {
@@ -263,9 +267,17 @@ __global__ void __launch_bounds__(kWideThreads, 1)
       int64_t g = 0;
       Ring<L::AST> r;
       bool ok = true;
+      ACursor<Tile> pc{walker, SET && a.prefetch > 0};
+      auto prefetch_next = [&]() {
+        if (!SET || !pc.next(n_tiles, n_walkers, decode)) return;
+#pragma unroll
+        for (int h = 0; h < 2 * KC / 32; h++) tma_prefetch_2d(&tmA, pc.kb * 2 * KC + 32 * h, pc.d.rowA);
+      };
+      for (int i = 0; SET && i < a.prefetch; i++) prefetch_next();
       for (int64_t t = walker; t < n_tiles && ok; t += n_walkers) {
         const Tile d = decode(t);
         for (int kb = d.kb0; kb < d.kb1; kb++, g++, r.next()) {
+          prefetch_next();
           const int s = r.s;
           if (g >= L::AST && !wait(&aempty[s], r.ph ^ 1)) {
             ok = false;
@@ -588,6 +600,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     const int q = warp & 3;
     const int row = q * 32 + lane;
     const int c0 = (e >> 2) * EC;
+    const bool streaming = !SET || (a.l2_mode & 2) != 0;  // C evict first
     uint8_t *buf0 = staging + e * 4096;
     wait_dependency();  // the column scales are written
     Ring<L::NACC> qe;
@@ -694,7 +707,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                 const int rr = 8 * u + (lane >> 2);
                 const uint4 w =
                     *reinterpret_cast<const uint4 *>(buf + rr * 64 + (((lane & 3) ^ ((rr >> 1) & 3)) << 4));
-                __stcs(reinterpret_cast<uint4 *>(a.C + om_u[u] + col), w);
+                store_c(reinterpret_cast<uint4 *>(a.C + om_u[u] + col), w, streaming);
               }
             }
           }
@@ -704,7 +717,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
           for (int j = 0; j < EC; j++) {
             if (j % 8 == 0) scale8(j);
             const int64_t col = __shfl_sync(0xffffffffu, off[j >> 5], j & 31);
-            if (n0 + j < a.N) __stcs(a.C + om + col, make_float2(re[j], im[j]));
+            if (n0 + j < a.N) store_c(a.C + om + col, make_float2(re[j], im[j]), streaming);
           }
         }
       } else if (a.tma_store) {
@@ -740,7 +753,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
               asm volatile(
                   "cp.async.bulk.tensor.2d.global.shared::cta.bulk_group.L2::cache_hint [%0, {%1, %2}], [%3], %4;" ::"l"(
                       (uint64_t)&tmC),
-                  "r"((int)(2 * (n0 + c))), "r"(y), "r"(smem_u32(buf)), "l"(l2_evict_first())
+                  "r"((int)(2 * (n0 + c))), "r"(y), "r"(smem_u32(buf)), "l"(streaming ? l2_evict_first() : l2_evict_normal())
                   : "memory");
               asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
@@ -751,7 +764,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
 #pragma unroll
         for (int j = 0; j < EC; j++) {
           if (j % 8 == 0) scale8(j);
-          if (n0 + j < a.N) __stcs(crow + n0 + j, make_float2(re[j], im[j]));
+          if (n0 + j < a.N) store_c(crow + n0 + j, make_float2(re[j], im[j]), streaming);
         }
       }
     }
