@@ -242,17 +242,18 @@ cudaError_t launch_direct(const DStep *steps, int n_steps, const int *bmap, int6
 // A run of small dependency levels in one launch: one cluster of CTAs (at
 // most eight) takes the levels one after the other, with a barrier of the
 // cluster between them, where a launch per level is bound by launch latency
-// (a replayed graph spends 3 to 4 us a level, whose work takes under one).
+// (a replayed graph spends about 2.5 us a level, whose work takes under one).
 // Work is dealt to warps, not blocks: small steps have a handful of outputs.
-// A warp task is 32 items of a step (output, part of the summed bits) or,
-// where a step sums over more than 32 parts, one output; parts are added in
-// the order of direct_block, so the results are bit-identical to it. A warp
-// reads its task of the next level before the barrier. Operands are read
+// A warp has at most one task in a level: 32 items of a step (output, part of
+// the summed bits), a few terms each (the plan chains no other levels). Parts are
+// added in the order of direct_block, so the results are bit-identical to it.
+// A warp reads its task of the next level before the barrier. Operands are read
 // through L2 where other CTAs wrote them a level before.
-// Bound by latency (dependent loads and the barrier, about 1.5 us a level): the
-// twelve levels of a 4 x 4 circuit of depth 10, 36 us as launches of a replayed
-// graph, take 20.7 us (whole call 73 -> 50 us, with the call's fewer launches
-// and copies); 24.9 us with descriptors fetched level by level.
+// Bound by latency (dependent loads and the barrier): a level takes about a
+// microsecond less than its launch, and the chain 1 to 2 us to start. The
+// twelve levels of at most 16 tasks of a 4 x 4 circuit of depth 10: 48.2 us a
+// call as launches, 36.0 in a chain of one CTA (42.2 in a cluster of two with
+// the level of 22 tasks before them).
 // tab: n_levels pairs (first task, tasks), then the tasks (step, number
 // within the step).
 constexpr int kChainThreads = 512, kChainWarps = kChainThreads / 32;
@@ -263,21 +264,12 @@ __device__ __forceinline__ void chain_task(const DStep &st, int sub, int lane, c
   const T *Bp = region_ptr<T>(st.B, cbase, abase);
   T *Cp = const_cast<T *>(region_ptr<T>(st.C, cbase, abase));
   const int split = st.split;
-  if (split <= 5) {
-    const int64_t item = (int64_t)sub * 32 + lane;
-    const int64_t c = item >> split;
-    const int part = (int)(item & ((1 << split) - 1));
-    const bool active = c < (int64_t(1) << st.nC);
-    const T sum = warp_parts(active ? direct_part<T, L2>(st, (uint32_t)c, part, Ap, Bp) : czero<T>(), split);
-    if (active && part == 0) Cp[c] = sum;
-  } else {
-    T sum = czero<T>();
-    for (int q = 0; q < (1 << (split - 5)); q++) {
-      const T v = direct_part<T, L2>(st, (uint32_t)sub, q * 32 + lane, Ap, Bp);
-      sum = q ? add_lanes(sum, v, 0, 32) : add_lanes(shfl_c(v, 0), v, 1, 31);
-    }
-    if (lane == 0) Cp[sub] = sum;
-  }
+  const int64_t item = (int64_t)sub * 32 + lane;
+  const int64_t c = item >> split;
+  const int part = (int)(item & ((1 << split) - 1));
+  const bool active = c < (int64_t(1) << st.nC);
+  const T sum = warp_parts(active ? direct_part<T, L2>(st, (uint32_t)c, part, Ap, Bp) : czero<T>(), split);
+  if (active && part == 0) Cp[c] = sum;
 }
 
 template <typename T>
@@ -289,7 +281,7 @@ __global__ void __launch_bounds__(kChainThreads) direct_chain_kernel(const DStep
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
   asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(ctas));
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  const int w = (int)rank * kChainWarps + warp, W = (int)ctas * kChainWarps;
+  const int w = (int)rank * kChainWarps + warp;
   // every level's bounds and every step's descriptor, read at once (fetched
   // level by level, each level waited for three dependent loads: 2.1 us a
   // level); a warp's task of the next level is read before the barrier
@@ -302,8 +294,7 @@ __global__ void __launch_bounds__(kChainThreads) direct_chain_kernel(const DStep
   for (int l = 0; l < n_levels; l++) {
     const int2 next = l + 1 < n_levels ? s_lv[l + 1] : make_int2(0, 0);
     const int2 ntask = w < next.y ? tasks[next.x + w] : make_int2(0, 0);
-    for (int t = w; t < lv.y; t += W) {
-      if (t != w) task = tasks[lv.x + t];
+    if (w < lv.y) {
       if (ctas == 1)
         chain_task<T, false>(s_st[task.x], task.y, lane, cbase, abase);
       else
@@ -319,10 +310,7 @@ __global__ void __launch_bounds__(kChainThreads) direct_chain_kernel(const DStep
   }
 }
 
-int chain_tasks(const DStep &st) {
-  if (st.split > 5) return 1 << st.nC;
-  return std::max(1, (1 << (st.nC + st.split)) / 32);
-}
+int chain_tasks(const DStep &st) { return std::max(1, (1 << (st.nC + st.split)) / 32); }
 
 int chain_ctas(int max_tasks) {
   int c = 1;
@@ -332,7 +320,7 @@ int chain_ctas(int max_tasks) {
 
 cudaError_t launch_direct_chain(const DStep *steps, int n_steps, const int *tab, int n_levels, int ctas,
                                 const char *cbase, char *abase, int dbl, cudaStream_t s) {
-  if (n_steps > kChainSteps || n_levels > kChainLevels) return cudaErrorInvalidValue;
+  if (n_steps > kChainSteps || n_levels > kChainLevels || ctas * kChainWarps > kChainTasks) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;

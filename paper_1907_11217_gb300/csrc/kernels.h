@@ -124,10 +124,10 @@ cudaError_t launch_direct(const DStep *steps, int n_steps, const int *bmap, int6
 // A run of small dependency levels in one launch (one cluster of at most
 // eight CTAs, a cluster barrier between levels); same results. steps: the
 // run's n_steps <= kChainSteps steps. tab (8-byte aligned): n_levels <=
-// kChainLevels pairs (first task, tasks), then the tasks as pairs (step,
-// number within the step). chain_tasks: warp tasks of a step; chain_ctas: CTAs
-// for levels of at most max_tasks tasks.
-constexpr int kChainSteps = 160, kChainLevels = 64;
+// kChainLevels pairs (first task, tasks <= kChainTasks: a warp each), then the
+// tasks as pairs (step, number within the step). chain_tasks: warp tasks of a
+// step with split <= 5; chain_ctas: CTAs for levels of at most max_tasks tasks.
+constexpr int kChainSteps = 160, kChainLevels = 64, kChainTasks = 128;
 int chain_tasks(const DStep &st);
 int chain_ctas(int max_tasks);
 cudaError_t launch_direct_chain(const DStep *steps, int n_steps, const int *tab, int n_levels, int ctas,

@@ -631,41 +631,78 @@ tz_plan *plan_create(const Network &net, const Pairs &pairs, const std::vector<i
       }
     }
   // ------------------------------------------------------- direct chains
-  // Consecutive small levels run as one launch: each at most kChainTasks
-  // warp tasks (two per warp of the largest cluster), so that a level takes
-  // less than the launch it replaces.
-  constexpr int kChainTasks = 256;
-  for (std::vector<Item> *items : {&p->var_items, &p->const_items})
-    for (size_t i = 0; i < items->size();) {
-      size_t j = i;
-      int most = 0;
-      while (j < items->size() && (*items)[j].kind == IT_DIRECT && !(*items)[j].queue) {
-        int64_t n = 0;
-        for (int d = (*items)[j].first; d < (*items)[j].first + (*items)[j].count && n <= kChainTasks; d++)
-          n += p->dsteps[d].nC > 20 ? kChainTasks + 1 : dev::chain_tasks(p->dsteps[d]);
-        const int steps = (*items)[j].first + (*items)[j].count - (*items)[i].first;
-        if (n > kChainTasks || steps > dev::kChainSteps || (int)(j - i) >= dev::kChainLevels) break;
-        most = std::max(most, (int)n);
-        j++;
+  // Consecutive small levels run as one launch where that saves time. A level
+  // may be part of a chain when every warp of the cluster has at most one task,
+  // of at most 16 terms (complex128: one, its units are few): longer sums are
+  // better spread over the chip (6 x 6 depth 24, four bitstrings: 147 us a call
+  // as launches, 224 with its level of 256 tasks of 128 terms in a chain).
+  // What a chain saves, fitted to 217 circuits of 3 x 4 to 6 x 6 (replayed
+  // graphs; us): it costs 2 to start on one CTA and 1 on a cluster, a level of
+  // it 1.1 or 0.8 less than a launch, 0.1 of which is lost with each doubling
+  // of the terms; in complex128 it saves 0.75 a level on one CTA and next to
+  // nothing on a cluster, which also starts in 2. The cheapest division of a run
+  // of such levels is taken, of chains that save a microsecond (the spread of the
+  // calls). Against launches alone no circuit then lost more than 3.4 %; by
+  // number of tasks alone (at most 256) one in five did, up to half its speed.
+  const bool dbl = p->esz == 16;
+  const double chain_start[2] = {2.0, dbl ? 2.0 : 1.0};  // [on a cluster]
+  const double chain_saves[2] = {dbl ? 0.75 : 1.1, dbl ? 0.1 : 0.8};
+  constexpr double kTermsCost = 0.1, kChainLeast = 1.0;
+  for (std::vector<Item> *items : {&p->var_items, &p->const_items}) {
+    auto level = [&](const Item &it) {  // (warp tasks, or 0: not part of a chain; log2 of a task's terms)
+      std::pair<int64_t, int> r(0, 0);
+      if (it.kind != IT_DIRECT || it.queue) return r;
+      for (int d = it.first; d < it.first + it.count; d++) {
+        const dev::DStep &ds = p->dsteps[d];
+        r.second = std::max(r.second, (int)ds.nK - (int)ds.split);
+        if (ds.split > 5 || ds.nC > 20) return std::pair<int64_t, int>(0, 0);
+        r.first += dev::chain_tasks(ds);
       }
-      if (j - i >= 2) {
-        Item &it = (*items)[i];
-        it.chain = (int)(j - i);
-        it.chain_ctas = dev::chain_ctas(most);
-        if (p->bmap.size() % 2) p->bmap.push_back(0);
-        it.chain_off = (int64_t)p->bmap.size() * 4;
-        std::vector<int32_t> levels, tasks;
-        for (size_t l = i; l < j; l++) {
-          levels.push_back((int32_t)tasks.size() / 2);
-          for (int d = (*items)[l].first; d < (*items)[l].first + (*items)[l].count; d++)
-            for (int t = 0; t < dev::chain_tasks(p->dsteps[d]); t++) tasks.insert(tasks.end(), {d - (*items)[i].first, t});
-          levels.push_back((int32_t)tasks.size() / 2 - levels.back());
+      if (r.first > dev::kChainTasks || r.second > (dbl ? 0 : 4)) r.first = 0;
+      return r;
+    };
+    const int n_items = (int)items->size();
+    std::vector<std::pair<int64_t, int>> lv(n_items);
+    std::vector<int> from(n_items + 1);
+    std::vector<double> best(n_items + 1, 0.0);  // cost against launches, the first j items divided best
+    for (int j = 1; j <= n_items; j++) {
+      best[j] = best[j - 1];
+      from[j] = j - 1;
+      lv[j - 1] = level((*items)[j - 1]);
+      int64_t most = 0;
+      int steps = 0, terms = 0;
+      for (int i = j - 1; i >= 0 && lv[i].first; i--) {
+        most = std::max(most, lv[i].first);
+        steps += (*items)[i].count;
+        terms += lv[i].second;
+        if (steps > dev::kChainSteps || j - i > dev::kChainLevels) break;
+        const bool cluster = dev::chain_ctas((int)most) > 1;
+        const double cost = chain_start[cluster] - (j - i) * chain_saves[cluster] + terms * kTermsCost;
+        if (cost <= -kChainLeast && best[i] + cost < best[j]) {
+          best[j] = best[i] + cost;
+          from[j] = i;
         }
-        p->bmap.insert(p->bmap.end(), levels.begin(), levels.end());
-        p->bmap.insert(p->bmap.end(), tasks.begin(), tasks.end());
       }
-      i = std::max(j, i + 1);
     }
+    for (int j = n_items; j > 0; j = from[j]) {
+      const int i = from[j];
+      if (j - i < 2) continue;
+      Item &it = (*items)[i];
+      it.chain = j - i;
+      it.chain_ctas = dev::chain_ctas((int)std::max_element(lv.begin() + i, lv.begin() + j)->first);
+      if (p->bmap.size() % 2) p->bmap.push_back(0);
+      it.chain_off = (int64_t)p->bmap.size() * 4;
+      std::vector<int32_t> levels, tasks;
+      for (int l = i; l < j; l++) {
+        levels.push_back((int32_t)tasks.size() / 2);
+        for (int d = (*items)[l].first; d < (*items)[l].first + (*items)[l].count; d++)
+          for (int t = 0; t < dev::chain_tasks(p->dsteps[d]); t++) tasks.insert(tasks.end(), {d - it.first, t});
+        levels.push_back((int32_t)tasks.size() / 2 - levels.back());
+      }
+      p->bmap.insert(p->bmap.end(), levels.begin(), levels.end());
+      p->bmap.insert(p->bmap.end(), tasks.begin(), tasks.end());
+    }
+  }
   // leaf jobs
   for (int l = 0; l < L; l++) {
     if (!p->T[l].var) continue;
@@ -838,7 +875,7 @@ std::string plan_describe(const tz_plan *p) {
     o << "[";
     for (size_t i = 0; i < v.size(); i++)
       o << (i ? "," : "") << "[" << v[i].kind << "," << v[i].a << "," << v[i].b << "," << v[i].first << ","
-        << v[i].count << "," << v[i].blocks << "," << (v[i].queue ? 1 : 0) << "]";
+        << v[i].count << "," << v[i].blocks << "," << (v[i].queue ? 1 : 0) << "," << v[i].chain << "]";
     o << "]";
   };
   o << "],\"dsteps\":[";
