@@ -487,7 +487,7 @@ struct TcSmem {
   static constexpr uint32_t A_COL0 = TMEM_COLS - ASLOTS * SLOT_COLS;
   static constexpr int NBUF = A_COL0 / ACC_COLS;
   static_assert(BNP <= 128, "an epilogue thread holds half a row of the tile in registers");
-  // barriers, then the TMEM address, the abort flag and two scale exponents
+  // barriers, then the TMEM address and the abort flag
   static_assert((3 * STAGES + 2 * NBUF + ASLOTS + 2 + XR) * 8 + 16 <= BARS, "barriers and flags fit in BARS");
   // the split warps run at most ASLOTS k-blocks ahead of the products, which
   // run at most NBUF ranges ahead of the epilogue: a split warp never reaches
@@ -1737,9 +1737,8 @@ static bool use_pairs(int precision, int64_t M, int64_t N, int pair) {
          tc_pair_supported(precision, M, N);
 }
 
-int cgemm_tc_launches(int precision, int64_t batch, int64_t M, int64_t N, int64_t K, bool scatter, int ksplit,
-                      int pair) {
-  const WidePlan w = wide_plan(precision, batch, M, N, K, scatter, ksplit, pair);
+int cgemm_tc_launches(int precision, int64_t batch, int64_t M, int64_t N, int64_t K, bool scatter, int ksplit) {
+  const WidePlan w = wide_plan(precision, batch, M, N, K, scatter, ksplit, -1);
   if (w.use) return 2 + (w.ks > 1 ? 1 : 0);
   return 2 + (precision == TZ_FP16X3 ? 1 : 0) +
          (!scatter && ksplit != 1 && split_k(precision, batch, M, N, K) > 1 ? 1 : 0);

@@ -1292,8 +1292,7 @@ static void autotune_tc_steps(tz_plan *p) {
     int c = it.chain ? 2 - it.chain : 1;
     if (it.kind == IT_GEMM && p->S[it.a].tc && !p->S[it.a].tc_simt) {
       const PStep &ps = p->S[it.a];
-      c = dev::cgemm_tc_launches(p->opts.precision, ps.batch, ps.M, ps.N, ps.K, !ps.row_major, ps.tc_ksplit,
-                                 ps.tc_pair);
+      c = dev::cgemm_tc_launches(p->opts.precision, ps.batch, ps.M, ps.N, ps.K, !ps.row_major, ps.tc_ksplit);
     } else if (it.kind == IT_ACCUM) {
       c = dev::accumulate_launches(p->net.batch_log2, p->net.n_open);
     }
