@@ -452,6 +452,14 @@ int tz_tune_preset(int precision, int64_t batch, int64_t m, int64_t n, int64_t k
 int tz_debug_stream_tile(int64_t batch, int64_t m, int64_t n, int64_t k, int scatter, const int8_t *pb,
                          const int8_t *pm, const int8_t *pn, int32_t *out, int *supported);
 
+/* Test hook (host only): how a tensor-core product of this shape runs, with
+ * the process-wide defaults; scatter: C written through a scatter map; ksplit
+ * and pair as a plan's step holds them (0 and -1: default). out (4 int32) =
+ * {1 wide (128-column) tiles, 0 narrow ones; CTAs per tile; K ranges; kernel
+ * launches}. TZ_EINVAL for shapes the mode does not take. */
+int tz_debug_tc_form(int precision, int64_t batch, int64_t m, int64_t n, int64_t k, int scatter, int ksplit, int pair,
+                     int32_t *out);
+
 /* Process-wide default of how the tensor-core products run where the shape
  * allows pairs (m a multiple of 256; 128-column tiles in split BF16 / FP16,
  * more than 64 columns in split TF32): 1 on pairs of CTAs on two SMs

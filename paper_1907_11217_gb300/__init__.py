@@ -28,6 +28,7 @@ __all__ = [
     "tz_contract_amplitudes_device", "tz_op_permute", "tz_op_cgemm", "tz_op_accumulate", "PRECISIONS",
     "tz_plan_status", "tz_op_cgemm_status", "tz_op_cgemm_static_status", "tz_debug_set_wait_limit",
     "tz_debug_stall_tensor_core", "tz_debug_stall_direct_queue", "tz_tune_tc_pairs", "tz_tune_tc_prefetch", "tz_debug_tune_force_simt", "tz_tune_preset", "tz_debug_stream_tile",
+    "tz_debug_tc_form",
     "TZ_C64_SIMT", "TZ_TF32X3", "TZ_BF16X3", "TZ_FP16X3",
 ]
 
@@ -377,6 +378,15 @@ def tz_debug_stream_tile(batch, m, n, k, pb=None, pm=None, pn=None):
     ranks = [(v[6 + 3 * r], v[7 + 3 * r], v[8 + 3 * r]) for r in range(16) if v[6 + 3 * r] >= 0]
     return {"bz": v[0], "bm": v[1], "bn": v[2], "nl": v[3], "kmax": v[4], "smem": v[5], "ranks": ranks,
             "lane_rank": v[54:86]}
+
+
+def tz_debug_tc_form(precision, batch, m, n, k, scatter=False, ksplit=0, pair=-1):
+    """Test hook (host only): how a tensor-core product runs, as a dict (wide
+    tiles or not, CTAs per tile, K ranges, kernel launches)."""
+    out = (ctypes.c_int32 * 4)()
+    check(lib().tz_debug_tc_form(PRECISIONS.get(precision, precision), int(batch), int(m), int(n), int(k),
+                                 int(bool(scatter)), int(ksplit), int(pair), ctypes.cast(out, ctypes.c_void_p)))
+    return {"wide": bool(out[0]), "ctas": out[1], "ksplit": out[2], "launches": out[3]}
 
 
 def tz_debug_tune_force_simt(on):

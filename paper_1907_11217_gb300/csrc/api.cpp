@@ -646,6 +646,20 @@ int tz_debug_stream_tile(int64_t batch, int64_t m, int64_t n, int64_t k, int sca
   TZ_CATCH
 }
 
+int tz_debug_tc_form(int precision, int64_t batch, int64_t m, int64_t n, int64_t k, int scatter, int ksplit, int pair,
+                     int32_t *out) {
+  TZ_TRY
+  REQUIRE(out, "NULL argument");
+  REQUIRE(batch >= 1 && m >= 1 && n >= 1 && k >= 1, "dimensions must be >= 1");
+  REQUIRE(tz::dev::cgemm_tc_supported(precision, m, n, k), "not a tensor-core product");
+  const tz::dev::TcForm f = tz::dev::cgemm_tc_form(precision, batch, m, n, k, scatter != 0, ksplit, pair);
+  out[0] = f.wide;
+  out[1] = f.ctas;
+  out[2] = f.ksplit;
+  out[3] = f.launches;
+  TZ_CATCH
+}
+
 int tz_debug_tune_force_simt(int on) {
   TZ_TRY
   tz::tune_force_simt(on);

@@ -1690,6 +1690,34 @@ struct WidePlan {
   int64_t Kp;      // K padded to whole k-blocks
   size_t half;     // bytes of the prepared hi (or lo) planes
 };
+// BF16 and TF32: whether wide tiles are quicker than narrow ones, twice as many
+// of half the columns. With fewer wide tiles than half the SMs they are not (32
+// of them, K = 1024: BF16 46 against 35 us, TF32 50 against 41; 128: 15.1 against
+// 16.6 and 15.3 against 17.9); with more, the tiles that the busiest CTA walks
+// decide (the last column tile is half empty for N = 129..192 and narrow tiles
+// fill the last wave better), against what a wide tile saves of the time of two
+// narrow ones: nothing in products of one k-block, which the stores bound,
+// 10 % from two k-blocks on, 15 % from ten, over 30 % from K = 512, and more
+// where B is large beside A (it is prepared in half the bytes). With rows of C
+// off 32 bytes wide tiles lose up to 20 % up to four k-blocks. Both forms over
+// 1248 shapes (N 66..1022, K 4..256), narrow against wide us: TF32 b16 M4096 N490
+// K16 66 against 81, b16 M4096 N160 K128 60 against 68, BF16 b16 M4096 N130 K64 33
+// against 42, b3 M2048 N512 K64 16.0 against 17.8; b16 M4096 N512 K256 188 against
+// 158 (TF32 258 against 233), b300 M256 N160 K128 84 against 77. The rule takes a
+// form 5 % or more slower than the other for 54 of them (303 by the number of
+// wide tiles alone) and loses 0.6 % on average (3.8 %).
+static bool wide_pays(int64_t row_tiles, int64_t M, int64_t N, int64_t K, int64_t kblocks) {
+  // (tiles of the busiest CTA; from eight narrow ones a CTA on, of the average)
+  const int64_t w = row_tiles * ((N + kWideCols - 1) / kWideCols), n = row_tiles * ((N + 63) / 64);
+  const bool many = n >= 8 * 152;
+  const double wide = many ? w / 152.0 : (double)((w + 151) / 152);
+  const double narrow = many ? n / 152.0 : (double)((n + 151) / 152);
+  double gain = kblocks < 2 ? 1.0 : kblocks < 10 ? 1.1 : K < 512 ? 1.15 : 1.34;
+  const double b = std::min(1.0, (double)N / (double)M);
+  if (kblocks >= 2) gain *= 1.0 + 0.5 * b;
+  if (N % 4 != 0 && kblocks <= 4) gain *= 0.8 + 0.2 * b;
+  return 2.0 * wide <= gain * narrow;
+}
 static WidePlan wide_plan(int precision, int64_t batch, int64_t M, int64_t N, int64_t K, bool scatter, int ksplit,
                           int pair) {
   WidePlan w{false, 1, 1, 0, 0};
@@ -1712,13 +1740,11 @@ static WidePlan wide_plan(int precision, int64_t batch, int64_t M, int64_t N, in
     const int room = split_k(precision, batch, M, N, K);
     w.ks = (int)std::max<int64_t>(1, std::min<int64_t>({room, 152 / std::max<int64_t>(tiles, 1), kblocks / 32}));
   }
-  // With fewer wide tiles than half the SMs the narrow form's twice as many
-  // CTAs win (32 wide tiles, K = 1024: BF16 46 against 35 us, TF32 50 against
-  // 41; 128 wide tiles: 15.1 against 16.6 and 15.3 against 17.9). FP16 takes
-  // them at any count: its one pass over B saves the launch and the read of a
-  // separate maximum (2 tiles 16.2 against 20.0 us, 32 tiles 24.9 against
-  // 26.9, 32 tiles of K = 1024 48.3 against 49.5).
-  w.use = precision == TZ_FP16X3 || tiles * w.ks >= 76;
+  // FP16 takes wide tiles at any count: its one pass over B saves the launch
+  // and the read of a separate maximum (2 tiles 16.2 against 20.0 us, 32 tiles
+  // 24.9 against 26.9, 32 tiles of K = 1024 48.3 against 49.5), and its split
+  // of A is the bound.
+  w.use = precision == TZ_FP16X3 || (tiles * w.ks >= 76 && (w.ks > 1 || wide_pays(batch * (M / BM), M, N, K, kblocks)));
   // Pairs: half of B per SM, so half of the shared-memory reads that the
   // products themselves make (64 of the 128 bytes a clock; the loads and the
   // split take another 63): BF16 M16384 N1024 K2048 466 -> 432 us, TF32 755 ->
@@ -1737,11 +1763,17 @@ static bool use_pairs(int precision, int64_t M, int64_t N, int pair) {
          tc_pair_supported(precision, M, N);
 }
 
-int cgemm_tc_launches(int precision, int64_t batch, int64_t M, int64_t N, int64_t K, bool scatter, int ksplit) {
-  const WidePlan w = wide_plan(precision, batch, M, N, K, scatter, ksplit, -1);
-  if (w.use) return 2 + (w.ks > 1 ? 1 : 0);
-  return 2 + (precision == TZ_FP16X3 ? 1 : 0) +
-         (!scatter && ksplit != 1 && split_k(precision, batch, M, N, K) > 1 ? 1 : 0);
+TcForm cgemm_tc_form(int precision, int64_t batch, int64_t M, int64_t N, int64_t K, bool scatter, int ksplit,
+                     int pair) {
+  const WidePlan w = wide_plan(precision, batch, M, N, K, scatter, ksplit, pair);
+  TcForm f{w.use, w.cg, w.ks, 2};
+  if (!w.use) {
+    f.ctas = use_pairs(precision, M, N, pair) ? 2 : 1;
+    f.ksplit = scatter || ksplit == 1 ? 1 : split_k(precision, batch, M, N, K);
+    if (precision == TZ_FP16X3) f.launches++;  // the maxima of |B|
+  }
+  if (f.ksplit > 1) f.launches++;
+  return f;
 }
 
 cudaError_t launch_cgemm_tc(int precision, const float2 *A, const float2 *B, float2 *C, int64_t batch, int64_t M,

@@ -212,10 +212,16 @@ cudaError_t tc_set_stall(int on);
 // for products that split K across CTAs the partial results, and in the FP16
 // mode the partial maxima of |B|.
 size_t cgemm_tc_scratch_bytes(int precision, int64_t batch, int64_t M, int64_t N, int64_t K);
-// Kernel launches of one tensor-core product (FP16 mode on narrow tiles: the
-// maxima of |B|; B preparation, the product, and the sum of split-K partials
-// when K is split; scatter outputs never split).
-int cgemm_tc_launches(int precision, int64_t batch, int64_t M, int64_t N, int64_t K, bool scatter, int ksplit = 0);
+// How launch_cgemm_tc runs a product (same arguments): wide or narrow tiles,
+// CTAs per tile, K ranges, and its kernel launches (B preparation and the
+// product; FP16 mode on narrow tiles: the maxima of |B|; the sum of split-K
+// partials when K is split; scatter outputs never split).
+struct TcForm {
+  bool wide;
+  int ctas, ksplit, launches;
+};
+TcForm cgemm_tc_form(int precision, int64_t batch, int64_t M, int64_t N, int64_t K, bool scatter, int ksplit = 0,
+                     int pair = -1);
 cudaError_t launch_accumulate(const AccumArgs &a, cudaStream_t s);
 // kernel launches of one launch_accumulate (2 when the root is too large for
 // one block: the group state then advances in a launch of its own)

@@ -819,7 +819,7 @@ tz_plan *plan_create(const Network &net, const Pairs &pairs, const std::vector<i
     if (it.kind == IT_GEMM) {
       const PStep &ps = p->S[it.a];
       if (ps.tc)
-        n = dev::cgemm_tc_launches(p->opts.precision, ps.batch, ps.M, ps.N, ps.K, !ps.row_major);
+        n = dev::cgemm_tc_form(p->opts.precision, ps.batch, ps.M, ps.N, ps.K, !ps.row_major).launches;
     } else if (it.kind == IT_ACCUM) {
       n = dev::accumulate_launches(net.batch_log2, net.n_open);
     }
@@ -1292,7 +1292,7 @@ static void autotune_tc_steps(tz_plan *p) {
     int c = it.chain ? 2 - it.chain : 1;
     if (it.kind == IT_GEMM && p->S[it.a].tc && !p->S[it.a].tc_simt) {
       const PStep &ps = p->S[it.a];
-      c = dev::cgemm_tc_launches(p->opts.precision, ps.batch, ps.M, ps.N, ps.K, !ps.row_major, ps.tc_ksplit);
+      c = dev::cgemm_tc_form(p->opts.precision, ps.batch, ps.M, ps.N, ps.K, !ps.row_major, ps.tc_ksplit).launches;
     } else if (it.kind == IT_ACCUM) {
       c = dev::accumulate_launches(p->net.batch_log2, p->net.n_open);
     }
