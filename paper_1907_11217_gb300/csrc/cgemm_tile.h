@@ -216,6 +216,11 @@ cudaError_t launch_tiled(const float2 *A, const float2 *B, float2 *C, int64_t ba
                          int64_t sA, int64_t sB, int64_t sC, const CScatter *sc, cudaStream_t s) {
   auto blocks = [&](int bm, int bn) { return ((M + bm - 1) / bm) * ((N + bn - 1) / bn) * batch; };
   if (N <= 4 && K > 8) return run_tile<64, 4, 4, 1, 16, 2, 4>(A, B, C, batch, M, N, K, sA, sB, sC, sc, s);
+  // few columns and a short sum (below 256 rows, where the skinny kernels start):
+  // bound by a tile's start and end, so no padded columns and a K tile of four
+  // (64 x 16 -> 64 x 4 tiles: b4096 M255 N2 K4 45 -> 16 us, b4096 M96 N1 K1 25 ->
+  // 10, b20000 M128 N2 K8 117 -> 62, 60 with a K tile of eight)
+  if (N <= 4 && M >= 64) return run_tile<64, 4, 4, 1, 4, 2, 4>(A, B, C, batch, M, N, K, sA, sB, sC, sc, s);
   if (N <= 16) {
     // few summed values: a short K tile, more rows a block
     if (K <= 8 && M >= 64) return run_tile<64, 16, 4, 2, 8, 2, 3>(A, B, C, batch, M, N, K, sA, sB, sC, sc, s);
