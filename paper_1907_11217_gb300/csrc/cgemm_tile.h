@@ -196,13 +196,24 @@ template <int BM, int BN, int TM, int TN, int BK, int NB, int MINB>
 cudaError_t run_tile(const float2 *A, const float2 *B, float2 *C, int64_t batch, int64_t M, int64_t N, int64_t K,
                      int64_t sA, int64_t sB, int64_t sC, const CScatter *sc, cudaStream_t s) {
   const int64_t mt = (M + BM - 1) / BM, nt = (N + BN - 1) / BN;
-  const int64_t blocks = (mt * nt * batch + NB - 1) / NB;
-  if (blocks > 0x7fffffff) return cudaErrorInvalidValue;
   const int vec = (K % 2) == 0 && (sA % 2) == 0 && (sB % 2) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0 &&
                   (reinterpret_cast<uintptr_t>(B) & 15) == 0;
   CScatter none{};
-  cgemm_tile_kernel<BM, BN, TM, TN, BK, NB, MINB><<<(unsigned)blocks, TileCfg<BM, BN, TM, TN, BK, NB>::NT, 0, s>>>(
-      A, B, C, batch, M, N, K, sA, sB, sC, sc ? *sc : none, sc ? 1 : 0, vec, mt, nt);
+  // A grid has at most 2^31 - 1 blocks: a batch of more tiles (of operands
+  // with strides of zero, say) goes in parts of 2^j products. (The first tile
+  // as a kernel argument cost every launch up to 6 %.)
+  int64_t part = batch;
+  if ((mt * nt * batch + NB - 1) / NB > 0x7fffffff) {
+    if (mt * nt > 0x7fffffff) return cudaErrorInvalidValue;
+    for (part = 1; 2 * part * mt * nt <= 0x7fffffff;) part *= 2;
+  }
+  for (int64_t z0 = 0; z0 < batch; z0 += part) {
+    const int64_t n = std::min(part, batch - z0);
+    cgemm_tile_kernel<BM, BN, TM, TN, BK, NB, MINB>
+        <<<(unsigned)((mt * nt * n + NB - 1) / NB), TileCfg<BM, BN, TM, TN, BK, NB>::NT, 0, s>>>(
+            A + z0 * sA, B + z0 * sB, C + (sc ? scatter_bits(z0, sc->nb, sc->pb) : z0 * sC), n, M, N, K, sA, sB, sC,
+            sc ? *sc : none, sc ? 1 : 0, vec, mt, nt);
+  }
   return cudaGetLastError();
 }
 

@@ -34,7 +34,7 @@ __device__ __forceinline__ T zero_c() {
   return z;
 }
 
-__device__ __forceinline__ int64_t scatter_bits(int64_t v, int n, const int8_t *pos) {
+__host__ __device__ __forceinline__ int64_t scatter_bits(int64_t v, int n, const int8_t *pos) {
   int64_t o = 0;
   for (int j = 0; j < n; j++) o |= ((v >> j) & 1) << pos[j];
   return o;
