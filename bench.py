@@ -211,12 +211,12 @@ def measured_peaks():
 
 
 # DRAM bytes (read + write) per tensor-core product launch, averaged over the
-# product launches of one step, from an ncu capture of the bench command itself
+# 13 product launches of one step, from an ncu capture of the bench command itself
 # with its autotuned choices fixed by --tune-file (dram__bytes_read.sum +
-# dram__bytes_write.sum, one pass), keyed by (precision, workload). A mode or
-# workload without a capture of the current kernels reports null; the launch
-# list under profiles/ is of the narrow product alone.
-TC_DRAM_BYTES_PER_LAUNCH = {}
+# dram__bytes_write.sum, one pass; profiles/launch_list_bristlecone70_d32_fp16x3.md),
+# keyed by (precision, workload). A mode or workload without a capture of the
+# current kernels reports null.
+TC_DRAM_BYTES_PER_LAUNCH = {("fp16x3", "bristlecone70_d32"): 1.8457e9}
 
 
 def plan_roofline(plan, precision, ms_per_group):
