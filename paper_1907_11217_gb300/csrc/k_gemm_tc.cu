@@ -1678,11 +1678,14 @@ int tc_l2_mode_default() {
 void tc_set_prefetch(int kblocks) { g_prefetch.store(kblocks < 0 ? -1 : std::min(64, kblocks), std::memory_order_relaxed); }
 
 // Wide tiles (tc_wide.h): whether a product takes them, and its K split.
-// Measured (2070 MHz limit, split FP16 / BF16 / TF32, before -> after):
+// Measured in runs of a few ms (2070 MHz limit, split FP16 / BF16 / TF32, before
+// -> after; under load for longer the power limit lowers the clock, and a call
+// of the FP16, TF32 and FP16 products below takes 640, 818 and 844 us):
 //   b8 M32768 N256 K512:   942 -> 551 us, 659 -> 494, 1014 -> 780
 //   b1 M16384 N1024 K2048: 940 -> 507 us (542 TF/s useful, 0.86 of the
 //     measured BF16 peak issued), 647 -> 432 (637, 1.01), 1036 -> 750
 //   b32 M512 N128 K16384:  1487 -> 795 us in FP16 (B prepared in half the bytes)
+// Which form BF16 and TF32 take: wide_pays() below.
 struct WidePlan {
   bool use;
   int cg;          // CTAs per tile: 2 (pairs, 256 rows) or 1

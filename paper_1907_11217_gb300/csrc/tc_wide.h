@@ -1,6 +1,6 @@
 // Wide-tile split-precision product (part of k_gemm_tc.cu: included inside
 // its anonymous namespace, after the PTX helpers). Products with more than
-// 64 complex columns and enough row tiles to fill the chip.
+// 64 complex columns; in BF16 and TF32 those for which wide_pays() says so.
 //
 // Tiles of 128 rows by 128 complex columns. Instead of one real product on
 // the interleaved view, the complex product is formed from its planes, four

@@ -24,7 +24,7 @@ def main():
     ap.add_argument("--iters", type=int, default=5)
     ap.add_argument("--warmup", type=int, default=2)
     ap.add_argument("--pairs", type=int, default=-1, choices=[-1, 0, 1],
-                    help="split BF16/FP16 products: 1 pairs of CTAs, 0 single CTAs, -1 default")
+                    help="tensor-core products: 1 pairs of CTAs where the shape allows, 0 single CTAs, -1 default")
     ap.add_argument("--prefetch", type=int, default=-1,
                     help="L2 prefetch distance of A tiles in k-blocks (0 off, -1 default)")
     a = ap.parse_args()
